@@ -10,10 +10,11 @@
 //   warps 0-3  softmax of tile A, warps 4-7 softmax of tile B: thread t owns
 //              row t & 127 of its tile. Per 128-key block it reads the 128
 //              scores from TMEM in two chunks of 64, exponentiates them
-//              against the row's reference (the max of the row's first block;
-//              raised only when a chunk's sum reaches 2^16), adds up the row
-//              sum and writes P (bf16) to the tile's TMEM P buffer. The S
-//              buffer is released as soon as both chunks have been loaded.
+//              against the row's reference (the max of the row's first chunk,
+//              raised when a later chunk's max exceeds it by more than 2^8),
+//              adds up the row sum and writes P (bf16) to the tile's TMEM P
+//              buffer. The S buffer is released as soon as both chunks have
+//              been loaded.
 //              Epilogue: O / l and the log-sum-exp to global (or page-locked
 //              host) memory, each row as four 32-byte stores, whole sectors;
 //   warps 8, 11  TMA producers: warp 8 the item queue, both query tiles (one
@@ -35,11 +36,11 @@
 // chunk body copied 1 / 3 / 6 times in straight line: 389 / 510 / 632 cycles per
 // chunk), and code run once costs about 5 cycles per instruction. So the code is kept small: one
 // rolled chunk body for every block, masks and maxima in a short loop over
-// TMEM that is called for an item's first and edge blocks only, the rare raise
-// out of line, and the warp index broadcast so that what depends on it stays in
+// TMEM that is called for an item's first and edge blocks only, the rare search
+// for a higher reference out of line, and the warp index broadcast so that what depends on it stays in
 // the uniform datapath. (Masks applied to the scores in registers also made the
 // compiler copy all 64 of them on the unmasked path.) Against the unrolled form
-// (73 KB of code, now 41): 256-row mixed batch 5300 -> 4565 us beside the
+// (73 KB of code, now 45): 256-row mixed batch 5300 -> 4565 us beside the
 // decode kernel, prefill of 8 prompts (35681 tokens, 1.61 TFLOP) 1677 -> 1475 us
 // = 1.09 PFLOP/s, window layer of 384 rows 250 -> 236 us. Measured slower:
 // four issuers (1737 us for the prefill), 16 softmax warps on key halves (1528),
@@ -86,11 +87,14 @@ constexpr uint32_t kTmemCols = 512;
 __device__ __forceinline__ uint32_t col_s(int x) { return x ? 128u : 0u; }
 __device__ __forceinline__ uint32_t col_o(int x) { return x ? 320u : 256u; }
 __device__ __forceinline__ uint32_t col_p(int x) { return x ? 448u : 384u; }
-// A chunk's sum of probabilities from which a row's reference is raised. Below
-// it nothing is rescaled: bf16 and fp32 keep their relative precision at any
-// scale. High enough that a reference taken over the few keys a row sees in its
-// first block (a window's) does not cause it.
-constexpr float kRaiseAt = 0x1p16f;
+// A row's reference is raised when a chunk's max exceeds it by more than
+// kRescaleThreshold (log2 units). A chunk whose sum is below 2^kRescaleThreshold
+// holds no such score, so only other chunks are searched for their max. The weights
+// that dominate a row then stand close to its reference, where a bf16 weight of
+// exactly 1 rounds nothing away: with a threshold of 2^16 the errors of full-context
+// rows grew by 8-12 % for scores of 4 and 16 times unit variance.
+constexpr float kRescaleThreshold = 8.f;
+constexpr float kSearchAt = 256.f;
 
 static_assert(kAppendTcRows == 2 * kTcRows, "an item is two tiles");
 
@@ -182,14 +186,16 @@ __device__ __forceinline__ bool wait_bar_poll(uint32_t bar, uint32_t parity, vol
 
 // A block with keys some row does not see, or without a reference yet: writes
 // -inf over the scores in TMEM (columns cS ..) of keys outside [lo, pos] and
-// returns the row's largest visible score (raw). A short loop, called once or
+// returns the largest visible score (raw) of the first 64 keys, or, if the row
+// sees none of them, of the others. A short loop, called once or
 // twice per item: the code that turns scores into probabilities stays the same
 // for every block, and small.
 __device__ __noinline__ float mask_block(uint32_t cS, int kb, int pos, int lo) {
-  float m0 = -INFINITY, m1 = -INFINITY;
+  float m0 = -INFINITY, m1 = -INFINITY, first = -INFINITY;
   const unsigned span = (unsigned)(pos - lo);
 #pragma unroll 1
   for (int c = 0; c < kTcKeys / 32; ++c) {
+    if (c == 2) first = fmaxf(m0, m1);
     uint32_t v[32];
     tmem_ld32(cS + 32 * c, v);
     tmem_ld_wait();
@@ -205,7 +211,7 @@ __device__ __noinline__ float mask_block(uint32_t cS, int kb, int pos, int lo) {
     tmem_st32(cS + 32 * c, v);
   }
   tmem_st_wait();
-  return fmaxf(m0, m1);
+  return first > -INFINITY ? first : fmaxf(m0, m1);
 }
 
 // The same for the short form, whose items are mostly such blocks. The warp's rows
@@ -215,13 +221,14 @@ __device__ __noinline__ float mask_block(uint32_t cS, int kb, int pos, int lo) {
 // want_max. A window layer of 384 rows: 238 -> 225.5 us. In the general form, where
 // it runs once or twice in an item of many blocks, it made a rollout step 1 % slower.
 __device__ __noinline__ float mask_block_short(uint32_t cS, int n, int kb, int pos, int lo, bool want_max) {
-  float m0 = -INFINITY, m1 = -INFINITY;
+  float m0 = -INFINITY, m1 = -INFINITY, first = -INFINITY;
   const unsigned span = (unsigned)(pos - lo);
   // keys that every row sees, and that some row sees
   const int all_lo = __reduce_max_sync(0xffffffffu, lo), all_hi = __reduce_min_sync(0xffffffffu, pos);
   const int any_lo = __reduce_min_sync(0xffffffffu, lo), any_hi = __reduce_max_sync(0xffffffffu, pos);
 #pragma unroll 1
   for (int c = 0; c < n; ++c) {
+    if (c == 2) first = fmaxf(m0, m1);
     uint32_t v[32];
     const int k0 = kb + 32 * c;
     const bool whole = k0 >= all_lo && k0 + 31 <= all_hi;
@@ -248,7 +255,7 @@ __device__ __noinline__ float mask_block_short(uint32_t cS, int n, int kb, int p
     }
   }
   tmem_st_wait();
-  return fmaxf(m0, m1);
+  return first > -INFINITY ? first : fmaxf(m0, m1);
 }
 
 // p = 2^(s * scale_log2 - m) for the 64 scores, packed to bf16 pairs; returns
@@ -275,6 +282,16 @@ __device__ __forceinline__ float chunk_exp(const uint32_t (&sv)[2][32], float sc
 __device__ __forceinline__ void st_shared_zero16(uint32_t addr) {
   asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(addr), "r"(0u) : "memory");
 }
+// 16 bytes of local memory (a: address in the local window)
+__device__ __forceinline__ void st_local_v4(uint32_t a, const uint32_t* w) {
+  asm volatile("st.local.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3])
+               : "memory");
+}
+__device__ __forceinline__ void ld_local_v4(uint32_t a, uint32_t* w) {
+  asm volatile("ld.local.v4.u32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
+               : "r"(a));
+}
 // one 32-byte store (p 32-byte aligned)
 __device__ __forceinline__ void st_global_v8(void* p, const uint32_t* w) {
   asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]),
@@ -296,66 +313,75 @@ __device__ __forceinline__ void selftest_stall(uint32_t never_bar, int32_t* abor
   atomicCAS(abort_flag, 0, 2);
 }
 
-// A chunk whose probabilities summed to kRaiseAt or more (or overflowed) in
-// some row of the warp: rare, so called and not inlined, and the scores come
-// through local memory. Such a row's reference is raised to the chunk's max,
-// its probabilities are computed again, and what was summed under the old
-// reference is rescaled: the earlier sums (factor alpha), this block's first
-// chunk of P (columns cP0, if fix_p) and O (columns cO, if fix_o). Writes the
-// chunk's P to columns cP. Whole warp.
-struct RaisedChunk {
-  float m_ref, sum, alpha;
-};
-__device__ __noinline__ RaisedChunk raise_chunk(const uint32_t* sv, float scale_log2, float m_ref, float sum,
-                                                uint32_t cP, uint32_t cP0, bool fix_p, uint32_t cO, bool fix_o) {
-  RaisedChunk r = {m_ref, sum, 1.f};
-  if (sum >= kRaiseAt) {
-    float mx = -INFINITY;
-#pragma unroll 1
-    for (int e = 0; e < 64; ++e) mx = fmaxf(mx, __uint_as_float(sv[e]) * scale_log2);
-    if (mx > m_ref) {
-      r.alpha = ex2_approx(m_ref - mx);
-      r.m_ref = mx;
+__device__ __forceinline__ float chunk_max(const uint32_t (&sv)[2][32]) {
+  float m0 = -INFINITY, m1 = -INFINITY;
+#pragma unroll
+  for (int c = 0; c < 2; ++c)
+#pragma unroll
+    for (int e = 0; e < 32; e += 4) {
+      m0 = fmax3(m0, __uint_as_float(sv[c][e]), __uint_as_float(sv[c][e + 1]));
+      m1 = fmax3(m1, __uint_as_float(sv[c][e + 2]), __uint_as_float(sv[c][e + 3]));
     }
+  return fmaxf(m0, m1);
+}
+
+// A chunk whose probabilities sum to kSearchAt or more (or overflow, or are NaN)
+// in some row of the warp: searched for its max, and where that exceeds the row's
+// reference by more than the threshold, the reference is raised to it. Writes the
+// chunk's P to columns cP, and rescales the block's first chunk of P (columns cP0)
+// if it is not this one. Called, not inlined: with this code in the chunk loop the
+// prefill of 8 prompts takes 1764 us instead of 1508. The scores are read from
+// columns cS, or, if S has been released, from local memory (`scores`). With scores
+// of 4 / 16 times unit variance, where most chunks of a warp raise some row, that
+// prefill takes 2347 / 2986 us; with all scores through local memory 2525 / 3471,
+// with S released only after the search 2181 / 2568 but 1801 at unit variance.
+struct SearchedChunk {
+  float m_ref, sum, alpha;  // alpha: factor of what was summed under the old reference
+};
+__device__ __noinline__ SearchedChunk search_chunk(uint32_t cS, bool released, uint32_t scores, float scale_log2,
+                                                   float m_ref, float sum, uint32_t cP, uint32_t cP0) {
+  SearchedChunk r = {m_ref, sum, 1.f};
+  uint32_t sv[2][32], pk[32];
+  if (!released) {
+    tmem_ld32(cS, sv[0]);
+    tmem_ld32(cS + 32, sv[1]);
+    tmem_ld_wait();
+  } else {
+#pragma unroll
+    for (int e = 0; e < 64; e += 4) ld_local_v4(scores + 4 * e, &sv[e >> 5][e & 31]);
+  }
+  const float mx = chunk_max(sv) * scale_log2;
+  if (!(sum < kSearchAt) && mx > m_ref + kRescaleThreshold) {
+    r.alpha = ex2_approx(m_ref - mx);
+    r.m_ref = mx;
   }
   __syncwarp();
-  r.sum = 0.f;
-  const float neg_mu = r.m_ref == -INFINITY ? 0.f : -r.m_ref;  // a row of the warp may see no key yet
-#pragma unroll 1
-  for (int c = 0; c < 4; ++c) {  // eight columns = 16 keys at a time
-    uint32_t pv[8];
+  r.sum = chunk_exp(sv, scale_log2, r.m_ref == -INFINITY ? 0.f : -r.m_ref, pk);
+  tmem_st32(cP, pk);
+  if (cP != cP0 && __any_sync(0xffffffffu, r.alpha != 1.f)) {
+    tmem_st_wait();
+    tmem_ld32(cP0, pk);
+    tmem_ld_wait();
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const float p0 = ex2_approx(fmaf(__uint_as_float(sv[16 * c + 2 * e]), scale_log2, neg_mu));
-      const float p1 = ex2_approx(fmaf(__uint_as_float(sv[16 * c + 2 * e + 1]), scale_log2, neg_mu));
-      r.sum += p0 + p1;
-      pv[e] = pack_bf16x2(p0, p1);
+    for (int e = 0; e < 32; ++e) {
+      const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&pk[e]));
+      pk[e] = pack_bf16x2(f.x * r.alpha, f.y * r.alpha);
     }
-    tmem_st8(cP + 8 * c, pv);
-    if (fix_p) {
-      tmem_st_wait();
-      tmem_ld8(cP0 + 8 * c, pv);
-      tmem_ld_wait();
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&pv[e]));
-        pv[e] = pack_bf16x2(f.x * r.alpha, f.y * r.alpha);
-      }
-      tmem_st8(cP0 + 8 * c, pv);
-    }
-  }
-  if (fix_o) {
-#pragma unroll 1
-    for (int c = 0; c < 8; ++c) {
-      uint32_t ov[8];
-      tmem_ld8(cO + 8 * c, ov);
-      tmem_ld_wait();
-#pragma unroll
-      for (int e = 0; e < 8; ++e) ov[e] = __float_as_uint(__uint_as_float(ov[e]) * r.alpha);
-      tmem_st8(cO + 8 * c, ov);
-    }
+    tmem_st32(cP0, pk);
   }
   return r;
+}
+// O (64 columns) times alpha. Whole warp.
+__device__ __noinline__ void rescale_o(uint32_t cO, float alpha) {
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h) {
+    uint32_t v[32];
+    tmem_ld32(cO + 32 * h, v);
+    tmem_ld_wait();
+#pragma unroll
+    for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) * alpha);
+    tmem_st32(cO + 32 * h, v);
+  }
 }
 
 }  // namespace
@@ -699,7 +725,8 @@ __global__ void __maxnreg__(144)
           const float mx = mask_block(cS, kb, pos, lo) * p.scale_log2;
           if (m_ref == -INFINITY) m_ref = mx;
         }
-        float lb = 0.f;
+        float lb = 0.f, alpha = 1.f;  // the block's sum; factor of what came before it
+        bool searched = false;
 #pragma unroll 1
         for (int c = 0; c < nc; ++c) {  // keys kb + 64c .. kb + 64c + 63
           uint32_t sv[2][32], pk[32];
@@ -718,21 +745,29 @@ __global__ void __maxnreg__(144)
             if (!ok) break;
             tc_fence_after();
           }
-          if (__any_sync(0xffffffffu, lc >= kRaiseAt)) {
-            uint32_t copy[64];
+          if (__any_sync(0xffffffffu, !(lc < kSearchAt))) {  // also for inf / NaN
+            uint4 copy[16];
+            const uint32_t scores = (uint32_t)__cvta_generic_to_local(copy);
+            if (c == nc - 1) {
 #pragma unroll
-            for (int e = 0; e < 32; ++e) copy[e] = sv[0][e], copy[32 + e] = sv[1][e];
-            const RaisedChunk r = raise_chunk(copy, p.scale_log2, m_ref, lc, cP + 32 * c, cP, c == 1, cO, b > 0);
+              for (int e = 0; e < 64; e += 4) st_local_v4(scores + 4 * e, &sv[e >> 5][e & 31]);
+            }
+            const SearchedChunk r =
+                search_chunk(cS + 64 * c, c == nc - 1, scores, p.scale_log2, m_ref, lc, cP + 32 * c, cP);
             m_ref = r.m_ref;
-            l *= r.alpha;
-            lb = lb * r.alpha + r.sum;
+            alpha *= r.alpha;
+            searched = true;
+            lb = __fmul_rn(lb, r.alpha);  // no fused multiply-add with the sum
+            lb += r.sum;
           } else {
             lb += lc;
             tmem_st32(cP + 32 * c, pk);
           }
         }
         if (!ok) break;
-        l += lb;
+        l = fmaf(l, alpha, lb);
+        // O_X may only be rescaled once PV_X(blk - 1) has completed (waited above)
+        if (b > 0 && searched && __any_sync(0xffffffffu, alpha != 1.f)) rescale_o(cO, alpha);
         // V rows of slots no query of the item sees (before key_begin on the
         // partial first page of a window, from key_end on the partial last
         // page) were perhaps never written and may hold NaN, which a zero

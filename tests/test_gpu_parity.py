@@ -98,10 +98,10 @@ def test_append_kernels_agree(seed):
 @pytest.mark.parametrize("g", [1, 8])
 @pytest.mark.parametrize("window", [0, 150])
 def test_append_references_that_rise(window, g):
-    # The append kernel exponentiates against the max of a row's first key
-    # block and raises it only when a 64-key chunk's sum reaches 2^16: keys
+    # The append kernel exponentiates against the max of a row's first 64 keys
+    # and raises it when a later 64-key chunk's max lies more than 2^8 above: keys
     # whose scores climb by 12 to 250 nats over the row (past 2^127 relative
-    # to the first block: probabilities overflow before the raise), in both
+    # to the first chunk: probabilities overflow before the raise), in both
     # chunks of a block, in single rows of a warp and in all of them.
     rng = np.random.default_rng(880 + window + g)
     b = W.build_batch("rising", 881 + g, [700, 300, 410], [300, 90, 33], 2 * g, 2, layer_windows=(window,))
@@ -118,6 +118,41 @@ def test_append_references_that_rise(window, g):
             elif j < S:  # one of the tokens the row appends
                 lay.k_new[int(b.query_start_loc[r]) + j - int(S - L)] = u * size
     _full_check(b, what=f"rising w{window} g{g}")
+
+
+@pytest.mark.parametrize("g", [1, 8])
+@pytest.mark.parametrize("window,low,high", [(0, 3, 100), (0, 3, 300), (200, 203, 270), (200, 203, 333)])
+def test_append_weight_that_dominates_is_not_rounded(window, low, high, g):
+    # A row whose first chunk's max is a key `low`, and a key `high` in a later
+    # chunk 2^11.5 to 2^15.8 above it (every other key 2^46 below): the reference
+    # is raised to `high`, whose bf16 weight is then exactly 1. What is left is the
+    # output's own rounding (2^-8 of it), and the bf16 rounding of the weight of
+    # `low` before and after it is rescaled: 2 x 2^-8 x 2^-11.5 x |v| < 1.5e-5; fp32
+    # sums add 2^-20 or so. A weight of 2^12.3 would be rounded by up to 2^-8 more.
+    S, L = 400, 40
+    b = W.build_batch("dominant", 890 + window + g, [S], [L], g, 1, layer_windows=(window,))
+    lay, pool = b.layers[0], b.pools[b.layers[0].pool]
+    f = torch.linspace(1.0, 1.37, L * g).view(L, g, 1).bfloat16()
+    lay.q[:] = f.expand(L, g, 64)
+    lay.k_new[:] = -4.0
+    at = torch.full((S - L,), -4.0)
+    at[low], at[high] = 0.0, 1.0
+    for j in range(S - L):
+        page = int(pool.block_table[0, j // 16])
+        if page >= 0:
+            pool.k_cache[page, :, j % 16] = at[j]
+    run, _ = _full_check(b, what="dominant")
+    kv = [W.to_host(x) for x in (run.kc, run.vc)]
+    first = 0 if window == 0 else S - L - window + 1
+    j = np.arange(first, S)
+    k, v = (oracle.bf16_bits_to_float(x)[pool.block_table[0, j // 16], 0, j % 16].astype(np.float64) for x in kv)
+    s = np.einsum("tgd,jd->tgj", lay.q.double().cpu().numpy(), k) * b.softmax_scale
+    pos = np.arange(S - L, S)[:, None, None]
+    s[np.broadcast_to((j > pos) | ((j <= pos - window) & (window > 0)), s.shape)] = -np.inf
+    p = np.exp(s - s.max(-1, keepdims=True))
+    ref = (p / p.sum(-1, keepdims=True)) @ v
+    err = np.abs(run.out_host()[0] - ref) - np.abs(ref) * 2.0 ** -8 * 1.001
+    assert err.max() <= 2e-5, err.max()
 
 
 @pytest.mark.parametrize("window", [0, 128])
