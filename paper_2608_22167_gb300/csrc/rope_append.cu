@@ -42,7 +42,11 @@ struct RopeParams {
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
 
-// Rotates 8 dims (x: dims i, y: dims i + 32) by the angles of cos c, sin s.
+// Rotates 8 dims (x: dims i, y: dims i + 32) by the angles of cos c, sin s. One
+// product of each sum is rounded to fp32, the other fused: which one is spelled
+// out, so that no compilation changes the last bit.
+__device__ __forceinline__ float rotate_lo(float a, float b, float c, float s) { return fmaf(a, c, -__fmul_rn(b, s)); }
+__device__ __forceinline__ float rotate_hi(float a, float b, float c, float s) { return fmaf(a, s, __fmul_rn(b, c)); }
 __device__ __forceinline__ void rotate8(uint4& x, uint4& y, const float (&c)[8], const float (&s)[8]) {
   uint32_t* xw = reinterpret_cast<uint32_t*>(&x);
   uint32_t* yw = reinterpret_cast<uint32_t*>(&y);
@@ -50,8 +54,8 @@ __device__ __forceinline__ void rotate8(uint4& x, uint4& y, const float (&c)[8],
   for (int i = 0; i < 4; ++i) {
     const float a0 = bf16_lo(xw[i]), a1 = bf16_hi(xw[i]), b0 = bf16_lo(yw[i]), b1 = bf16_hi(yw[i]);
     const float c0 = c[2 * i], c1 = c[2 * i + 1], s0 = s[2 * i], s1 = s[2 * i + 1];
-    xw[i] = pack_bf16x2(a0 * c0 - b0 * s0, a1 * c1 - b1 * s1);
-    yw[i] = pack_bf16x2(b0 * c0 + a0 * s0, b1 * c1 + a1 * s1);
+    xw[i] = pack_bf16x2(rotate_lo(a0, b0, c0, s0), rotate_lo(a1, b1, c1, s1));
+    yw[i] = pack_bf16x2(rotate_hi(a0, b0, c0, s0), rotate_hi(a1, b1, c1, s1));
   }
 }
 

@@ -75,6 +75,29 @@ def test_rope_kv_append_matches_the_oracle(seed):
     assert_parity(got_out, got_lse, oracle.bf16_bits_to_float(ref_out), ref_lse, "after rope append")
 
 
+def test_rotation_rounds_as_stated():
+    # y_i = fma(x_i, c, -[x_{i+32} s]) and y_{i+32} = fma(x_i, s, [x_{i+32} c]) in
+    # fp32, then bf16, bit for bit. In 64 bits a product of bf16 and fp32 is exact,
+    # and so is the sum for operands of like size; 4 million values, of which the
+    # other choice of the fused product changes one in fifty thousand.
+    T, H = 4096, 16
+    gen = torch.Generator("cuda").manual_seed(520)
+    q, k, v = (torch.randn(T, n, 64, generator=gen, device="cuda").bfloat16() for n in (H, 2, 2))
+    tab = torch.from_numpy(W.rope_table(T)).cuda()
+    kc, vc = (torch.zeros(T // 16, 2, 16, 64, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    bt = torch.arange(T // 16, dtype=torch.int32, device="cuda")[None]
+    one = lambda *x: torch.tensor(x, dtype=torch.int32, device="cuda")  # noqa: E731
+    status = one(0)
+    got = q.clone()
+    mcpu.mcpu_rope_kv_append(got, k, v, kc, vc, bt, one(T), one(0, T), tab, status)
+    assert int(status) == 0
+    c, s = tab[:, None, :32].double(), tab[:, None, 32:].double()
+    for x, y in ((q, got), (k, kc.transpose(1, 2).reshape(T, 2, 64))):
+        a, b = x[..., :32].double(), x[..., 32:].double()
+        lo, hi = a * c - (b * s).float().double(), a * s + (b * c).float().double()
+        assert torch.equal(y, torch.cat([lo, hi], -1).float().bfloat16())
+
+
 def test_rope_positions_past_the_table_are_reported():
     b = W.build_batch("ropebad", 520, [40, 300], [1, 20], 16, 2)
     run = Run(b)
