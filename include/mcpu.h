@@ -77,7 +77,8 @@ typedef enum mcpu_status {
   MCPU_ERR_WORKSPACE_TOO_SMALL = 3,  /* workspace_bytes < mcpu_workspace_size(dims) */
   MCPU_ERR_CUDA = 4,                 /* a CUDA runtime call failed (launch, attributes) */
   MCPU_ERR_BAD_PAGE = 5,             /* device: a needed block-table entry is outside the pool */
-  MCPU_ERR_BAD_LENGTHS = 6,          /* device: L_r > S_r, L_r < 0, S_r beyond the table, or
+  MCPU_ERR_BAD_LENGTHS = 6,          /* device: L_r > S_r, L_r < 0, S_r beyond the table, a row's
+                                        tokens outside [0, total_q), or
                                         query_start_loc[0] != 0 / [B] != total_q */
   MCPU_ERR_TIMEOUT = 7,              /* device: a bounded wait gave up */
   MCPU_ERR_INTERNAL = 8,             /* device: work plan overflowed its bound */

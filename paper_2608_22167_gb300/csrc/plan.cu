@@ -182,7 +182,8 @@ __global__ void __launch_bounds__(NT, 1) plan_kernel(AttnParams p) {
       const int q0 = p.qsl[r], q1 = p.qsl[r + 1], s = p.seq_lens[r];
       if ((r == 0 && q0 != 0) || (r == B - 1 && q1 != p.total_q)) bad_global = 1;
       const int len = q1 - q0;
-      const bool bad = len < 0 || s < len || s > p.max_pages * kPage;
+      // a row's tokens lie in [0, total_q): every kernel after this one trusts its record's token
+      const bool bad = q0 < 0 || q1 > p.total_q || len < 0 || s < len || s > p.max_pages * kPage;
       // decode-only calls (fp8 pools) report and skip append rows
       const bool skip = !bad && p.decode_only && len > 1;
       if (bad) status |= kStatusBadLengths;

@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 import oracle
 
 if torch.cuda.is_available():
-    from _gpu import Run, assert_parity, oracle_full, oracle_sampled
+    from _gpu import Run, assert_parity, from_fp8_blocks, oracle_full, oracle_sampled
     from paper_2608_22167_gb300 import mcpu
 
 
@@ -578,6 +578,65 @@ def test_inconsistent_lengths_are_reported():
     code, bits = run2.status()
     assert code == 6 and bits & mcpu.STATUS_BAD_LENGTHS
     assert run2.header()["n_decode"] == 0 and run2.header()["n_append"] == 0
+
+
+@pytest.mark.parametrize("kv", ["bf16", "mma_sync", "fp8"])
+@pytest.mark.parametrize("qsl,good", [
+    ([0, 100, 50, 60], [2]),          # row 0 runs past the last token
+    ([0, -5, 10, 60], [2]),           # an append row that starts before the first
+    ([0, 61, 62, 59, 60], [3]),       # a decode row behind the last token
+    ([0, -3, -2, 1, 2, 60], [3, 4]),  # a decode row before the first
+    ([0, 6, 7, -1, 0, 1, 1, 2], [4, 6]),  # both, in a call with fewer tokens than rows
+])
+def test_rows_outside_the_batch_are_reported_and_left_alone(qsl, good, kv):
+    # query_start_loc from 0 to total_q, but not monotone: rows whose tokens lie
+    # outside [0, total_q) are skipped. q, out and lse sit inside larger tensors
+    # whose rows around them must keep what they hold.
+    B, T, pad, Hq, Hkv, P = len(qsl) - 1, qsl[-1], 128, 16, 2, 160
+    if kv == "fp8" and T > B:
+        pytest.skip("fp8 calls take at most one token per row")
+    rng = np.random.default_rng(78 + B)
+    S = rng.integers(150, 300, size=B).astype(np.int32)
+    gen = torch.Generator("cuda").manual_seed(78)
+    normal = lambda *n: torch.randn(n, generator=gen, device="cuda").bfloat16()  # noqa: E731
+    q_all, kc, vc = normal(T + 2 * pad, Hq, 64), normal(P, Hkv, 16, 64), normal(P, Hkv, 16, 64)
+    out_all = torch.full_like(q_all, 7.0)
+    lse_all = torch.full((T + 2 * pad, Hq), 7.0, device="cuda")
+    q, out, lse = (x[pad:pad + T] for x in (q_all, out_all, lse_all))
+    bt_h = rng.permutation(P)[:19 * B].reshape(B, 19).astype(np.int32)
+    bt, sl, qs = (torch.from_numpy(np.asarray(x, np.int32)).cuda() for x in (bt_h, S, qsl))
+    scale = 64 ** -0.5
+    if kv == "fp8":
+        kv8 = mcpu.new_fp8_pool(P, Hkv)
+        at = torch.arange(P + 1, dtype=torch.int32, device="cuda")
+        token_major = lambda x: x.transpose(1, 2).reshape(P * 16, Hkv, 64).contiguous()  # noqa: E731
+        ws = mcpu.new_workspace(mcpu.dims_fp8(q, kv8, bt, sl))
+        mcpu.mcpu_kv_append_fp8(token_major(kc), token_major(vc), kv8, at[:P].view(P, 1), torch.full_like(at[:P], 16),
+                                at * 16, mcpu.status_word(ws))
+        assert mcpu.mcpu_read_device_status(ws)[0] == 0
+        mcpu.mcpu_paged_attention_forward_fp8(q, kv8, bt, sl, qs, 0, scale, out, lse, ws)
+    else:
+        ws = mcpu.new_workspace(mcpu.dims(q, kc, bt, sl))
+        mcpu.mcpu_paged_attention_forward(q, kc, vc, bt, sl, qs, 0, scale, out, lse, ws,
+                                          flags=mcpu.FLAG_MMA_SYNC_APPEND if kv == "mma_sync" else 0)
+    code, bits = mcpu.mcpu_read_device_status(ws)
+    assert code == 6 and bits & mcpu.STATUS_BAD_LENGTHS, (code, bits)
+    written = torch.zeros(T, dtype=torch.bool, device="cuda")
+    for r in good:
+        a, b = qsl[r], qsl[r + 1]
+        written[a:b] = True
+        args = (W.to_host(q[a:b]), W.to_host(kc), W.to_host(vc), bt_h[r:r + 1], S[r:r + 1],
+                np.array([0, b - a], np.int32), 0, scale)
+        if kv == "fp8":
+            pools = from_fp8_blocks(kv8.cpu().numpy())
+            ref, ref_lse = oracle.paged_attention_fp8(args[0], *pools, *args[3:])
+        else:
+            ref, ref_lse = oracle.paged_attention(*args)
+        assert_parity(out[a:b].float().cpu().numpy(), lse[a:b].cpu().numpy(), oracle.bf16_bits_to_float(ref), ref_lse,
+                      f"row {r}")
+    for x, y in ((out_all, out), (lse_all, lse)):
+        assert (x[:pad] == 7).all() and (x[pad + T:] == 7).all(), "written outside the batch"
+        assert (y[~written] == 7).all(), "a skipped row was written"
 
 
 def test_largest_row_count():
