@@ -167,7 +167,7 @@ mcpu_status mcpu_kv_append(const void* k_new, const void* v_new, void* k_cache, 
  * append kernel: the call forks it and the merge onto a library-owned,
  * low-priority stream of the current device after the planner and joins back
  * at the end, with CUDA events. Pass MCPU_FLAG_SERIAL to keep every kernel on
- * `stream`; a call with no more tokens than rows keeps them there too. out and
+ * `stream`; a call with as many tokens as rows keeps them there too. out and
  * lse may be page-locked host memory the device can address: out is written in
  * 32-byte pieces (whole sectors, if out is 32-byte aligned), which the host
  * link takes far better than halves of sectors. The call is capturable in a CUDA graph (with mcpu_kv_append

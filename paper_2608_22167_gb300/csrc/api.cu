@@ -350,15 +350,21 @@ mcpu_status mcpu_paged_attention_forward(const void* q, const void* k_cache, con
     if (r == cudaSuccess) r = mark(3, on);
     return r;
   };
-  // No more tokens than rows: a decode step (an append row would need empty
-  // rows beside it). Everything goes in one chain of programmatic launches,
-  // each grid launched while the one before it runs: the append kernel, which
-  // finds no work, the decode kernel, the merge. Against the fork below (two
-  // event records and waits, ordinary launches): 4 short rows 20.6 -> 18.4 us, 384
-  // windowed rows 36.0 -> 35.5, 64 rows of up to 16k keys 197 -> 194. With more
-  // tokens than rows the fork is better: the merge runs beside the append
-  // kernel (256 mixed rows 4925 us, as a chain 5013).
-  const bool chain = pdl && !serial && !legacy_append && p.total_q <= p.num_seqs;
+  // As many tokens as rows: a decode step (an append row would need empty rows
+  // beside it). Everything goes in one chain of programmatic launches, each grid
+  // launched while the one before it runs: the append kernel, which finds no
+  // work, the decode kernel, the merge. Every grid waits for the one before it
+  // before it reads anything that an earlier one wrote: only that wait makes it
+  // visible. Against the fork below (two event records and waits, ordinary
+  // launches): 4 short rows 20.6 -> 18.5 us, 384 windowed rows 36.0 -> 35.5, 64
+  // rows of up to 16k keys 197 -> 194. If there are append rows after all, the
+  // decode kernel comes after the append kernel, not beside it: 40 decode rows
+  // and a chunk of 217 tokens in 256 slots 142 -> 236 us. So calls with fewer
+  // tokens than rows (empty rows, perhaps chunks) take the fork: 156 decode rows
+  // of 256 slots 402 us either way, with a chunk of 90 tokens 406 against 518. So
+  // do those with more tokens: the merge then runs beside the append kernel (256
+  // mixed rows 4925 us, as a chain 5013).
+  const bool chain = pdl && !serial && !legacy_append && p.total_q == p.num_seqs;
   p.chained = chain;
   cudaError_t e = mark(0, s);
   if (e == cudaSuccess) e = launch_plan(p, s, pdl);
@@ -480,13 +486,19 @@ mcpu_status mcpu_paged_attention_forward_fp8(const void* q, const void* kv8, con
   };
   const bool cascade = p.cascade_enabled && p.window == 0;
   // every kernel on `stream`: there is no append kernel to run beside; they are
-  // programmatic launches unless phase events are recorded between them
+  // programmatic launches unless phase events are recorded between them. The
+  // decode kernel is one only if no cascade pass follows: that pass reads the plan
+  // without waiting for the decode kernel, whose tail it fills, and so needs the
+  // planner to have ended before the decode kernel began. (Waiting instead: 16
+  // groups of 8 rows 328 -> 337 us, 48 groups 976 -> 998; the ordinary launch costs
+  // an eager call about 2.5 us, 64 rows of up to 16k keys 123.0 -> 125.5, and a
+  // replayed graph 0.5.)
   const bool pdl = ev == nullptr;
-  p.chained = pdl;
+  p.chained = pdl && !cascade;
   cudaError_t e = mark(0);
   if (e == cudaSuccess) e = launch_plan(p, s, pdl);
   if (e == cudaSuccess) e = mark(1);
-  if (e == cudaSuccess) e = launch_decode_fp8(kv8, p, dev->sms * dev->bpsm_fp8, false, s, pdl);
+  if (e == cudaSuccess) e = launch_decode_fp8(kv8, p, dev->sms * dev->bpsm_fp8, false, s, p.chained);
   if (e == cudaSuccess) e = mark(2);
   if (e == cudaSuccess && cascade)
     e = launch_decode_fp8(kv8, p, dev->sms * dev->bpsm_fp8_cascade, true, s, pdl);

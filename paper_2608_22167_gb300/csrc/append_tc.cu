@@ -392,8 +392,9 @@ __global__ void __maxnreg__(144)
     append_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
                      const __grid_constant__ CUtensorMap qmap, const AttnParams p) {
   // launched programmatically (a call that may have decode rows only): wait for
-  // the planner's records, then let the decode kernel launch beside. Without
-  // the condition the kernel's main loop ran 1.5 % slower in every other call.
+  // the planner's records, then let the decode kernel be launched (it waits for
+  // this grid). Without the condition the kernel's main loop ran 1.5 % slower in
+  // every other call.
   if (p.chained) {
     grid_dep_wait();
     grid_dep_launch();

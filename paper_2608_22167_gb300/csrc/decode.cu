@@ -367,6 +367,9 @@ template <int KINDS>
 __global__ void __launch_bounds__(kDecodeWarps * 32, 5)
     decode_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
                   const AttnParams p) {
+  // In a chain of programmatic launches the plan is visible, and the grid
+  // before this one complete, only after this wait.
+  if (p.chained) grid_dep_wait();
   extern __shared__ uint8_t smem_raw[];
   const bool cascade = (KINDS & kKindCascade) && header(p)->n_cascade > 0;
   const bool decode = (KINDS & kKindDecode) && header(p)->n_decode > 0;
@@ -393,9 +396,6 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 5)
   }
   // no item left for this warp: the grid after this one may launch
   grid_dep_launch();
-  // In a chain of programmatic launches this grid's end implies the end of the
-  // one before it (the merge comes after both): its first CTA waits for that.
-  if (blockIdx.x == 0) grid_dep_wait();
 }
 
 using DecodeKernel = void (*)(const CUtensorMap, const CUtensorMap, const AttnParams);
@@ -403,8 +403,7 @@ constexpr DecodeKernel kDecodeKernels[] = {decode_kernel<kKindDecode>, decode_ke
                                            decode_kernel<kKindDecode | kKindCascade>};
 
 // `kinds`: kKindDecode, kKindCascade or both. `programmatic`: launched with
-// programmatic stream serialization after a kernel that has itself waited for
-// the planner.
+// programmatic stream serialization (p.chained set).
 cudaError_t launch_decode(const CUtensorMap& kmap, const CUtensorMap& vmap, const AttnParams& p, int grid, int kinds,
                           cudaStream_t stream, bool programmatic) {
   LaunchCfg lc(dim3(grid), dim3(kDecodeWarps * 32), decode_smem_bytes(), stream, programmatic);

@@ -97,10 +97,11 @@ __device__ __forceinline__ uint32_t key_byte_mask(int c, int lo, int hi) {
 template <int NT>
 __global__ void __launch_bounds__(kF8Warps * 32, NT == 1 ? 4 : 3)
     decode_fp8_kernel(const uint8_t* __restrict__ kv8, const AttnParams p) {
-  // Programmatic launches: the decode kernel waits for the planner; the cascade
-  // pass after it, which reads nothing that the decode kernel writes, does not,
-  // but its first CTA waits for that kernel before it exits, so that the
-  // pass's end implies the decode kernel's (the merge comes after both).
+  // Programmatic launches: the decode kernel waits for the planner. The cascade
+  // pass reads nothing that the decode kernel before it writes, and the planner
+  // ended before that kernel, an ordinary launch then, began: it does not wait,
+  // but its first CTA does before it exits, so that the pass's end implies the
+  // decode kernel's (the merge comes after both).
   if (NT == 1) grid_dep_wait();
   if ((NT == 1 ? header(p)->n_decode : header(p)->n_cascade) == 0) {  // nothing of this kind
     if (NT > 1 && blockIdx.x == 0) grid_dep_wait();
@@ -580,7 +581,8 @@ cudaError_t launch_kv_append_fp8(const void* k_new, const void* v_new, void* kv8
 }
 
 // `programmatic`: launched with programmatic stream serialization, the decode
-// kernel right after the planner, the cascade pass right after the decode kernel.
+// kernel right after the planner, the cascade pass right after the decode kernel
+// (itself an ordinary launch).
 cudaError_t launch_decode_fp8(const void* kv8, const AttnParams& p, int grid, bool cascade, cudaStream_t stream,
                               bool programmatic) {
   const uint8_t* pool = static_cast<const uint8_t*>(kv8);

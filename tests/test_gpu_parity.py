@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 import oracle
 
 if torch.cuda.is_available():
-    from _gpu import Run, assert_parity, from_fp8_blocks, oracle_full, oracle_sampled
+    from _gpu import Fp8Run, Run, assert_parity, from_fp8_blocks, oracle_full, oracle_sampled
     from paper_2608_22167_gb300 import mcpu
 
 
@@ -654,12 +654,59 @@ def test_largest_row_count():
     _good_rows_parity(run, b, rows, "2048 rows")
 
 
+@pytest.mark.parametrize("kv", ["bf16", "fp8"])
+@pytest.mark.parametrize("window", [0, 100, 300])
+def test_replayed_decode_steps_follow_new_lengths_and_tables(window, kv):
+    # A decode step captured once (one chain of programmatic launches), replayed
+    # back to back while seq_lens and the block table change: every kernel of a
+    # replay has to see that replay's plan. Rows change places, so that shared
+    # prefixes come and go, rows are split in some replays and not in others.
+    rng = np.random.default_rng(95 + window)
+    B, G = 24, 8
+    grp = np.arange(B) // G
+    prompt = np.array([900, 40, 2000])[grp]
+    S = (prompt + rng.integers(300, 1500, size=B)).astype(np.int32)
+    b = W.build_batch("replay", 96, S, np.ones(B, np.int64), 16, 2, shared_prefix_pages=prompt // 16,
+                      prompt_lens=prompt, group_of_row=grp)  # without a window: every page is allocated
+    run = Fp8Run(b) if kv == "fp8" else Run(b)
+    run.window = window
+    run.append()
+    run.forward()
+    assert run.status()[0] == 0
+    bt0 = run.bt.clone()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        run.forward()
+    steps = []
+    for i in range(8):
+        perm = np.arange(B) if i % 3 == 0 else rng.permutation(B)
+        sl = np.maximum(S - rng.integers(0, [2, 300, 1200][i % 3], size=B), 1).astype(np.int32)[perm]
+        steps.append([perm, sl, torch.from_numpy(perm).cuda(), torch.from_numpy(sl).cuda()])
+    torch.cuda.synchronize()
+    for step in steps:  # nothing waits for the device in between
+        run.bt.copy_(bt0[step[2]])
+        run.sl.copy_(step[3])
+        g.replay()
+        step += [run.out.clone(), run.lse.clone()]
+    assert run.status()[0] == 0
+    q, bt_h = W.to_host(run.q), bt0.cpu().numpy()
+    for i, (perm, sl, _, _, out, lse) in enumerate(steps):
+        args = (bt_h[perm], sl, b.query_start_loc, window, b.softmax_scale)
+        if kv == "fp8":
+            ref, ref_lse = oracle.paged_attention_fp8(q, *run.pools_host(), *args)
+        else:
+            ref, ref_lse = oracle.paged_attention(q, W.to_host(run.kc), W.to_host(run.vc), *args)
+        assert_parity(out.float().cpu().numpy(), lse.cpu().numpy(), oracle.bf16_bits_to_float(ref), ref_lse,
+                      f"replay {i}")
+
+
 @pytest.mark.parametrize("layer", [0, 1])
 def test_programmatic_launches_match_ordinary_ones_bitwise(layer):
-    # Without phase events the planner (after the prefix scan), the cascade
-    # pass (after the decode kernel) and the merge (after the cascade pass)
-    # are programmatic launches that overlap the grid before them; with phase
-    # events every kernel is an ordinary launch. Layer 1 of the rollout
+    # Without phase events the planner (after the prefix scan) and the merge
+    # (after the decode kernel) are programmatic launches that overlap the grid
+    # before them, and in a call with as many tokens as rows all kernels but the
+    # first; with phase events every kernel is an ordinary launch, and the decode
+    # items and the cascade items have one each. Layer 1 of the rollout
     # profiling batch has GRPO groups (cascade items) and split rows; layer 0
     # is a sliding-window layer. Results must agree bit for bit, eagerly and
     # as a replayed CUDA graph of the programmatic form.

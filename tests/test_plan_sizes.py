@@ -1,6 +1,6 @@
 """The planner's forms at the row counts where they change, cascade subgroups
 at the edges of an item's 16 query vectors, the launch order taken when a call
-has no more tokens than rows, the merge at the part counts where it spreads a
+has as many tokens as rows, the merge at the part counts where it spreads a
 row over more warps, windows at the size up to which rows are not split, and
 append items that end on half a block of keys (GPU, against the oracle)."""
 from __future__ import annotations
@@ -52,15 +52,15 @@ def test_cascade_subgroups(g, size):
     assert _check(b)["n_cascade"] >= 2 * -(-size * g // 16)
 
 
-@pytest.mark.parametrize("extra", [0, 1])
+@pytest.mark.parametrize("extra", [-1, 0, 1])
 @pytest.mark.parametrize("window", [0, 100])
 @pytest.mark.parametrize("n_app", [0, 1, 5])
-def test_as_many_tokens_as_rows_or_one_more(n_app, window, extra):
+def test_as_many_tokens_as_rows_or_one_more_or_less(n_app, window, extra):
     # append rows beside empty ones: with as many tokens as rows the kernels go
-    # in one chain, with one more in the fork; both equal the serial order
+    # in one chain, else in the fork; both equal the serial order
     from paper_2608_22167_gb300 import mcpu
 
-    rng = np.random.default_rng(100 * n_app + window + extra)
+    rng = np.random.default_rng(100 * n_app + window + extra + 1)
     B = 48
     L = np.ones(B, np.int64)
     L[2:2 + n_app] = 7
