@@ -334,21 +334,33 @@ __device__ __forceinline__ float chunk_max(const uint32_t (&sv)[2][32]) {
 // columns cS, or, if S has been released, from local memory (`scores`). With scores
 // of 4 / 16 times unit variance, where most chunks of a warp raise some row, that
 // prefill takes 2347 / 2986 us; with all scores through local memory 2525 / 3471,
-// with S released only after the search 2181 / 2568 but 1801 at unit variance.
+// with S released only after the search 2181 / 2568 but 1801 at unit variance. The
+// short form's items are a few blocks long, and its code the better for being
+// shorter: always through local memory, by plain accesses (a window layer of 384
+// rows 209.6 -> 207.0 us; in the general form plain ones made the prefill 1508 -> 1534).
 struct SearchedChunk {
   float m_ref, sum, alpha;  // alpha: factor of what was summed under the old reference
 };
-__device__ __noinline__ SearchedChunk search_chunk(uint32_t cS, bool released, uint32_t scores, float scale_log2,
+template <bool kShort, typename Scores>  // uint4*, or an address in the local window
+__device__ __noinline__ SearchedChunk search_chunk(uint32_t cS, bool released, Scores scores, float scale_log2,
                                                    float m_ref, float sum, uint32_t cP, uint32_t cP0) {
   SearchedChunk r = {m_ref, sum, 1.f};
   uint32_t sv[2][32], pk[32];
-  if (!released) {
+  if (!kShort && !released) {
     tmem_ld32(cS, sv[0]);
     tmem_ld32(cS + 32, sv[1]);
     tmem_ld_wait();
   } else {
 #pragma unroll
-    for (int e = 0; e < 64; e += 4) ld_local_v4(scores + 4 * e, &sv[e >> 5][e & 31]);
+    for (int e = 0; e < 64; e += 4) {
+      if constexpr (kShort) {
+        const uint4 v = scores[e / 4];
+        uint32_t* at = &sv[e >> 5][e & 31];
+        at[0] = v.x, at[1] = v.y, at[2] = v.z, at[3] = v.w;
+      } else {
+        ld_local_v4(scores + 4 * e, &sv[e >> 5][e & 31]);
+      }
+    }
   }
   const float mx = chunk_max(sv) * scale_log2;
   if (!(sum < kSearchAt) && mx > m_ref + kRescaleThreshold) {
@@ -748,13 +760,23 @@ __global__ void __maxnreg__(144)
           }
           if (__any_sync(0xffffffffu, !(lc < kSearchAt))) {  // also for inf / NaN
             uint4 copy[16];
-            const uint32_t scores = (uint32_t)__cvta_generic_to_local(copy);
-            if (c == nc - 1) {
+            SearchedChunk r;
+            if constexpr (kShort) {
 #pragma unroll
-              for (int e = 0; e < 64; e += 4) st_local_v4(scores + 4 * e, &sv[e >> 5][e & 31]);
+              for (int e = 0; e < 16; ++e) {
+                const uint32_t* v = &sv[e >> 3][4 * (e & 7)];
+                copy[e] = make_uint4(v[0], v[1], v[2], v[3]);
+              }
+              r = search_chunk<true, const uint4*>(cS + 64 * c, true, copy, p.scale_log2, m_ref, lc, cP + 32 * c, cP);
+            } else {
+              const uint32_t scores = (uint32_t)__cvta_generic_to_local(copy);
+              if (c == nc - 1) {
+#pragma unroll
+                for (int e = 0; e < 64; e += 4) st_local_v4(scores + 4 * e, &sv[e >> 5][e & 31]);
+              }
+              r = search_chunk<false, uint32_t>(cS + 64 * c, c == nc - 1, scores, p.scale_log2, m_ref, lc, cP + 32 * c,
+                                                cP);
             }
-            const SearchedChunk r =
-                search_chunk(cS + 64 * c, c == nc - 1, scores, p.scale_log2, m_ref, lc, cP + 32 * c, cP);
             m_ref = r.m_ref;
             alpha *= r.alpha;
             searched = true;
