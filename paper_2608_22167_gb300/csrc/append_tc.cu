@@ -72,9 +72,14 @@ namespace mcpu {
 
 constexpr int kTcRows = 128;                          // rows per tile (TMEM lanes)
 constexpr int kTcKeys = 128;                          // keys per block
-// Ring depths and the register cap leave room on every SM for one CTA of the
-// memory-bound decode kernel (side stream): 145 KiB of shared memory here,
-// and 3 warps x 144 registers on each SM sub-partition.
+// Ring depths and registers leave room on every SM for one CTA of the
+// memory-bound decode kernel (side stream): 145 KiB of shared memory here, and 3
+// warps x 136 registers on each SM sub-partition of 512, which leaves 104 for the
+// decode kernel's warp (96). The kernel takes 134; a test holds both to that sum.
+// Its own cap is 144 all the same: capped at 136 the compiler takes 128 and a
+// slower schedule (prefill of 8 prompts 1508 -> 1767 us). With no room for the
+// decode CTA its work follows the append kernel's: a form of this kernel that took
+// 144 registers lost 1700 us of the mixed batch's 4923 and 350 of the prefill's 1508.
 constexpr int kTcKStages = 4, kTcVStages = 3;
 constexpr int kTcQBytes = kAppendTcRows * kRowBytes;  // both tiles: 32 KiB
 constexpr int kTcTileQBytes = kTcRows * kRowBytes;    // 16 KiB
