@@ -38,7 +38,6 @@ struct PlanSmem {
   int n_own[kMaxSeqs];       // decode records
   int item_off[kMaxSeqs];    // first decode record
   int slot0[kMaxSeqs];       // partial slot of the row's first own split
-  int n_cs[kMaxSeqs];        // cascade splits covering the row
   int sg_off[kMaxSeqs];      // first cascade record (subgroup-first rows)
   int gs[kMaxSeqs];          // first row of the row's run (group)
   int mrank[kMaxSeqs];       // members in the rows before
@@ -46,7 +45,6 @@ struct PlanSmem {
   int grp_ndec[kMaxSeqs];    // per group, at its first row: decode rows
   int app_row[kMaxSeqs];     // append rows, longest first
   int app_off[kMaxSeqs];     // first append record of the row of that rank
-  unsigned char flags[kMaxSeqs];
   int warp_max[32];          // warp totals of the scans
   int warp_sum[6][32];
   int total_wm, total_wlb;
@@ -413,8 +411,6 @@ __global__ void __launch_bounds__(NT, 1) plan_kernel(AttnParams p) {
       o_rows += 1 << 16;
     }
     if (tot_cascade > 0) {
-      sm.flags[r] = (unsigned char)flags[i];
-      sm.n_cs[r] = n_cs[i];
       sm.sg_off[r] = o_sg;
       if (flags[i] & kFlagSubFirst) o_sg += n_cs[i];
     }
