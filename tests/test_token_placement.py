@@ -8,6 +8,7 @@ import pytest
 import torch
 
 import workloads as W
+from _gpu import to_fp8_blocks
 from paper_2608_22167_gb300 import mcpu
 
 pytestmark = pytest.mark.gpu
@@ -51,12 +52,20 @@ def test_every_token_lands_in_its_slot(B, hkv):
     mcpu.mcpu_kv_append(k, v, kc, vc, bt, sl, qsl, st)
     assert torch.equal(kc, placed(k)) and torch.equal(vc, placed(v))
 
-    # one token per call of the fp8 append over zeroed blocks: K codes and scales
+    # the fp8 append over zeroed blocks: K and V codes and scales, whole blocks
+    # (slots of no token stay zero)
     kv8 = torch.zeros(P, hkv, 2176, dtype=torch.uint8, device="cuda")
     mcpu.mcpu_kv_append_fp8(k, v, kv8, bt, sl, qsl, st)
-    a = k.float().abs().amax(-1, keepdim=True)
-    codes = (k.float() * (torch.full_like(a, 448.0) / a)).to(torch.float8_e4m3fn).view(torch.uint8)
-    assert torch.equal(kv8[..., :1024].reshape(P, hkv, 16, 64), placed(codes))
+    codes, scales = [], []
+    for x in (k, v):
+        a = x.float().abs().amax(-1, keepdim=True)
+        top = torch.full_like(a, 448.0)
+        codes.append(placed((x.float() * (top / a)).to(torch.float8_e4m3fn).view(torch.uint8)))
+        pool = torch.zeros(P * 16, hkv, device="cuda")
+        pool[dst] = (a / top)[..., 0]
+        scales.append(pool.view(P, 16, hkv).transpose(1, 2))
+    want = to_fp8_blocks(*(x.cpu().numpy() for x in codes + scales))
+    assert np.array_equal(kv8.cpu().numpy(), want)
 
     # RoPE: q in place for a head count that leaves a partial step of eight
     # rows, cos/sin table both 16-byte aligned and not
