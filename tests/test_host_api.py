@@ -127,11 +127,11 @@ def test_direct_outputs_equal_the_staged_ones_bitwise(pinned):
 @pytest.mark.parametrize("window", [0, 100])
 @pytest.mark.parametrize("hq,hkv", [(64, 8), (32, 8), (16, 8), (8, 8)])
 def test_forward_into_host_memory_equals_device_outputs_bitwise(hq, hkv, window):
-    # MCPU_FLAG_HOST_OUT_DIRECT on a forward call: out and lse are page-locked
-    # host memory, and the append kernel writes each row as four 32-byte
-    # stores (eight 16-byte ones when out is only 16-byte aligned, the second
-    # buffer here): g = 8, 4, 2, 1 and partial last tiles. The values are
-    # those of the device-output form, bit for bit.
+    # out and lse of a forward call in page-locked host memory: the append kernel
+    # writes each row as four 32-byte stores (eight 16-byte ones when out is only
+    # 16-byte aligned, the second buffer here): g = 8, 4, 2, 1 and partial last
+    # tiles. The values are those of device outputs, bit for bit, with
+    # MCPU_FLAG_HOST_OUT_DIRECT, which changes nothing on a forward call.
     seq = np.array([900, 40, 2500, 16, 700, 333, 77])
     ql = np.array([1, 17, 300, 1, 45, 333, 5])
     b = W.build_batch("host_out", 3400 + hq + window, seq, ql, hq, hkv, layer_windows=(window,))
@@ -162,7 +162,7 @@ def test_forward_into_host_memory_equals_device_outputs_bitwise(hq, hkv, window)
         assert code == 0, bits
         assert torch.equal(out_h.view(torch.int16), out_d.cpu().view(torch.int16)), off
         assert torch.equal(lse_h, lse_d.cpu()), off
-    if hq == 64:  # the device-output form is checked against the oracle elsewhere for every g
+    if hq == 64:  # device outputs are checked against the oracle elsewhere for every g
         ref_out, ref_lse = oracle_full(b, 0)[:2]
         assert_parity(out_h.float().numpy(), lse_h.numpy(), ref_out, ref_lse, f"host outputs W={window}")
 
