@@ -343,10 +343,11 @@ mcpu_status mcpu_paged_attention_forward(const void* q, const void* k_cache, con
   // events each kind has a launch of its own, the decode items' first.
   auto launch_decode_kernel = [&](cudaStream_t on, bool programmatic) -> cudaError_t {
     const int grid = dev->sms * dev->bpsm_decode;
-    if (!ev) return launch_decode(kmap, vmap, p, grid, kKindDecode | (cascade ? kKindCascade : 0), on, programmatic);
+    const int kind_cascade = kKindCascade | (p.wide_cascade ? kKindWide : 0);
+    if (!ev) return launch_decode(kmap, vmap, p, grid, kKindDecode | (cascade ? kind_cascade : 0), on, programmatic);
     cudaError_t r = launch_decode(kmap, vmap, p, grid, kKindDecode, on, false);
     if (r == cudaSuccess) r = mark(2, on);
-    if (r == cudaSuccess && cascade) r = launch_decode(kmap, vmap, p, grid, kKindCascade, on, false);
+    if (r == cudaSuccess && cascade) r = launch_decode(kmap, vmap, p, grid, kind_cascade, on, false);
     if (r == cudaSuccess) r = mark(3, on);
     return r;
   };
@@ -366,6 +367,8 @@ mcpu_status mcpu_paged_attention_forward(const void* q, const void* k_cache, con
   // mixed rows 4925 us, as a chain 5013).
   const bool chain = pdl && !serial && !legacy_append && p.total_q == p.num_seqs;
   p.chained = chain;
+  // a decode step has no append kernel for the cascade pass to run beside
+  p.wide_cascade = cascade && p.total_q == p.num_seqs;
   cudaError_t e = mark(0, s);
   if (e == cudaSuccess) e = launch_plan(p, s, pdl);
   if (e == cudaSuccess) e = mark(1, s);

@@ -29,6 +29,14 @@ constexpr int kMinSharedPages = 4;    // shortest prefix worth a cascade pass
 // -> 16: 48 groups of 8 with appending rows 6341 -> 6181 us per layer (the pass
 // no longer follows the append kernel), 16 groups of 8 638 -> 610 us.
 constexpr int kCascadeVectors = 16;
+// Where nothing runs beside the pass (calls with as many tokens as rows), items of
+// twice as many vectors (168 registers, as many CTAs: shared memory bounds them) read
+// L2 half as often, and pay once there are enough of them: from kWidePages pages of
+// 16-vector items per warp. 16 -> 32 vectors, H_q / H_kv = 64 / 8, own contexts of
+// up to 300 keys: 48 groups of 8 with prompts of 4-8 thousand tokens 262 -> 210 us
+// (320 pages per warp), 6 groups of 8 with 4000 51.2 -> 45.1 (26); but 4 groups of 8
+// with 4000 36.9 -> 41.1 (17.5), one of 8 with 8000 32.9 -> 39.0 (9).
+constexpr int kWidePages = 24;
 constexpr int kAppendRowsMin = 64;    // smallest append tile (query rows = tokens x heads)
 constexpr int kAppendTcRows = 256;    // query rows of one tcgen05 append item (two 128-row tiles)
 
@@ -82,7 +90,8 @@ struct PlanHeader {
   int32_t append_ticket; // dynamic scheduler counters, reset by the planner
   int32_t decode_ticket;
   int32_t cascade_ticket;
-  int32_t pad[54];
+  int32_t cascade_wide;  // 1: cascade items hold up to 2 * kCascadeVectors query vectors
+  int32_t pad[53];
 };
 static_assert(sizeof(PlanHeader) == 256, "header is one 256-byte block");
 
@@ -118,7 +127,8 @@ __host__ __device__ inline WorkspaceLayout workspace_layout(int32_t num_seqs, in
   return w;
 }
 
-constexpr int kKindDecode = 1, kKindCascade = 2;  // items a decode launch takes
+// Items a decode launch takes; kKindWide: cascade items may be wide ones
+constexpr int kKindDecode = 1, kKindCascade = 2, kKindWide = 4;
 
 // Arguments every attention kernel receives (by value).
 struct AttnParams {
@@ -142,6 +152,7 @@ struct AttnParams {
   const float* sinks;            // [Hq] sink logits (natural log), or null
   int32_t decode_only;           // 1: rows with L > 1 are reported and skipped (fp8 pools)
   int32_t chained = 0;           // 1: the kernel after the planner is a programmatic launch
+  int32_t wide_cascade = 0;      // 1: the planner may choose wide cascade items
   // read only by the self-test form of the append kernel: the role that
   // stalls and the report it writes (mcpu_selftest_append_abort)
   int32_t selftest_stall = -1;

@@ -3,7 +3,7 @@
 // One warp owns one work item: a contiguous range of pages of one kv head,
 // for either one decode row (NT = 1: its g <= 8 query heads) or a cascade
 // subgroup (NT = 2: up to 16 query vectors = members x g heads, all reading
-// the same shared prompt pages once). Per page the warp
+// the same shared prompt pages once; NT = 4: up to 32). Per page the warp
 //   - receives the 2 KiB K block and 2 KiB V block of (page, kv head) from a
 //     per-warp ring of kDecodeStages stages filled by 2-D TMA loads (128-byte
 //     swizzle, so ldmatrix reads are bank-conflict free);
@@ -364,7 +364,7 @@ __device__ __forceinline__ bool decode_items(const CUtensorMap& kmap, const CUte
 // on a sub-partition of 512 x 32 registers leave 104); shared memory alone
 // allows three CTAs beside one another.
 template <int KINDS>
-__global__ void __launch_bounds__(kDecodeWarps * 32, 5)
+__global__ void __launch_bounds__(kDecodeWarps * 32, (KINDS & kKindWide) ? 3 : 5)
     decode_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
                   const AttnParams p) {
   // In a chain of programmatic launches the plan is visible, and the grid
@@ -391,7 +391,12 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 5)
     }
     __syncwarp();
     bool ok = true;
-    if (cascade) ok = decode_items<kCascadeVectors / 8>(kmap, vmap, p, w);
+    if (cascade) {
+      if ((KINDS & kKindWide) && header(p)->cascade_wide)
+        ok = decode_items<2 * kCascadeVectors / 8>(kmap, vmap, p, w);
+      else
+        ok = decode_items<kCascadeVectors / 8>(kmap, vmap, p, w);
+    }
     if (decode && ok) decode_items<1>(kmap, vmap, p, w);
   }
   // no item left for this warp: the grid after this one may launch
@@ -399,20 +404,23 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 5)
 }
 
 using DecodeKernel = void (*)(const CUtensorMap, const CUtensorMap, const AttnParams);
-constexpr DecodeKernel kDecodeKernels[] = {decode_kernel<kKindDecode>, decode_kernel<kKindCascade>,
-                                           decode_kernel<kKindDecode | kKindCascade>};
+constexpr DecodeKernel kDecodeKernels[] = {  // by kinds
+    nullptr, decode_kernel<kKindDecode>, decode_kernel<kKindCascade>, decode_kernel<kKindDecode | kKindCascade>,
+    nullptr, nullptr, decode_kernel<kKindCascade | kKindWide>, decode_kernel<kKindDecode | kKindCascade | kKindWide>};
 
-// `kinds`: kKindDecode, kKindCascade or both. `programmatic`: launched with
+// `kinds`: kKindDecode, kKindCascade or both, kKindWide with kKindCascade if
+// p.wide_cascade is set. `programmatic`: launched with
 // programmatic stream serialization (p.chained set).
 cudaError_t launch_decode(const CUtensorMap& kmap, const CUtensorMap& vmap, const AttnParams& p, int grid, int kinds,
                           cudaStream_t stream, bool programmatic) {
   LaunchCfg lc(dim3(grid), dim3(kDecodeWarps * 32), decode_smem_bytes(), stream, programmatic);
-  return cudaLaunchKernelEx(&lc.cfg, kDecodeKernels[kinds - 1], kmap, vmap, p);
+  return cudaLaunchKernelEx(&lc.cfg, kDecodeKernels[kinds], kmap, vmap, p);
 }
 
 cudaError_t prepare_decode_kernels(int* blocks_per_sm) {
-  *blocks_per_sm = 1 << 20;  // the least of the three (shared memory: the same for all)
+  *blocks_per_sm = 1 << 20;  // the least of all (shared memory: the same for all)
   for (DecodeKernel k : kDecodeKernels) {
+    if (k == nullptr) continue;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)decode_smem_bytes());
     if (e != cudaSuccess) return e;
     // the same (largest) shared-memory carveout as the append kernel, so that

@@ -48,6 +48,7 @@ struct PlanSmem {
   int warp_max[32];          // warp totals of the scans
   int warp_sum[6][32];
   int total_wm, total_wlb;
+  int cascade_pages;         // pages of all cascade items of kCascadeVectors vectors
 };
 
 namespace {
@@ -156,13 +157,14 @@ __global__ void __launch_bounds__(NT, 1) plan_kernel(AttnParams p) {
   PlanHeader* hdr = header(p);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int B = p.num_seqs;
-  const int sub_cap = kCascadeVectors / p.group;  // rows per cascade item
+  int sub_cap = kCascadeVectors / p.group;  // rows per cascade item
   auto publish = [&](int n_decode, int n_cascade, int n_append, int n_merge, int n_parts) {
     hdr->n_decode = n_decode;
     hdr->n_cascade = n_cascade;
     hdr->n_append = n_append;
     hdr->n_merge = n_merge;
     hdr->n_parts = n_parts;
+    hdr->cascade_wide = sub_cap > kCascadeVectors / p.group;
     hdr->append_ticket = hdr->decode_ticket = hdr->cascade_ticket = 0;
   };
 
@@ -171,7 +173,7 @@ __global__ void __launch_bounds__(NT, 1) plan_kernel(AttnParams p) {
   // ---- phase 1: per-row kind (0 none / invalid, 1 decode, 2 append) and lengths
   int S[R], L[R], Q0[R], kind[R];
   int status = 0, bad_global = 0;
-  if (tid == 0) sm.total_wm = sm.total_wlb = 0;
+  if (tid == 0) sm.total_wm = sm.total_wlb = sm.cascade_pages = 0;
 #pragma unroll
   for (int i = 0; i < R; ++i) {
     const int r = tid * R + i;
@@ -271,8 +273,12 @@ __global__ void __launch_bounds__(NT, 1) plan_kernel(AttnParams p) {
         mr[i] = rank;
         if (r < B) sm.mrank[r] = rank;
         rank += m[i];
+        if (r < B && gs[i] == r && sm.grp_ndec[r] >= 2 && sm.grp_pages[r] >= kMinSharedPages)
+          atomicAdd(&sm.cascade_pages, sm.grp_pages[r] * cdiv(sm.grp_ndec[r], sub_cap));
       }
       __syncthreads();
+      if (p.wide_cascade && (long long)sm.cascade_pages * p.num_kv_heads > (long long)kWidePages * p.total_warps_hint)
+        sub_cap *= 2;
 #pragma unroll
       for (int i = 0; i < R; ++i) {
         if (!m[i]) continue;

@@ -7,6 +7,7 @@ from __future__ import annotations
 
 import numpy as np
 import pytest
+import torch
 
 import workloads as W
 from _gpu import Run, assert_parity, oracle_full
@@ -50,6 +51,45 @@ def test_cascade_subgroups(g, size):
     b = W.build_batch(f"sub{g}_{size}", 10 * g + size, S, np.ones(B, np.int64), 2 * g, 2,
                       shared_prefix_pages=prompt // 16, prompt_lens=prompt, group_of_row=grp)
     assert _check(b)["n_cascade"] >= 2 * -(-size * g // 16)
+
+
+@pytest.mark.parametrize("heads,size,prompt", [(64, 24, 4000), (64, 25, 4010), (64, 47, 2100), (32, 45, 4100),
+                                               (16, 67, 5700), (8, 177, 4040)])
+def test_wide_cascade_items(heads, size, prompt):
+    # decode steps with enough shared pages take cascade items of 32 query vectors
+    # (full and partial ones), the same with phase events or on one stream; a group
+    # of two rows and a row of no group beside
+    from paper_2608_22167_gb300 import mcpu
+
+    rng = np.random.default_rng(size)
+    g, grp = heads // 8, np.r_[np.zeros(size, int), np.ones(size, int), 2, 2, -1]
+    pr = np.r_[np.full(size, prompt), np.full(size, prompt + 64), 100, 100, 0]
+    S = pr + rng.integers(1, 60, size=2 * size + 3)
+    b = W.build_batch(f"wide{heads}_{size}", size, S, np.ones(S.size, np.int64), heads, 8, shared_prefix_pages=pr // 16,
+                      prompt_lens=pr, group_of_row=grp)
+    run = Run(b)
+    run.append()
+    run.forward()
+    assert run.status()[0] == 0
+    assert int(run.ws[40:44].view(torch.int32)) == 1  # header: wide items
+    C, subs = run.header()["split_pages"], -(-size // (32 // g))
+    splits = [-(-(p // 16) // C) for p in (prompt, prompt + 64, 100)]
+    assert run.header()["n_cascade"] == subs * (splits[0] + splits[1]) + splits[2]
+    one = run.out_host()
+    ref_out, ref_lse, _ = oracle_full(b)
+    assert_parity(*one, ref_out, ref_lse, b.name)
+    for kw in (dict(flags=mcpu.FLAG_SERIAL), "events"):
+        run.out.fill_(float("nan"))
+        if kw == "events":
+            ev = [torch.cuda.Event(enable_timing=True) for _ in range(mcpu.NUM_PHASE_EVENTS)]
+            for e in ev:  # torch creates the CUDA event at its first record
+                e.record()
+            mcpu.mcpu_paged_attention_forward(run.q, run.kc, run.vc, run.bt, run.sl, run.qsl, 0, b.softmax_scale,
+                                              run.out, run.lse, run.ws, phase_events=ev)
+        else:
+            run.forward(**kw)
+        for x, y in zip(one, run.out_host()):
+            assert np.array_equal(x, y)
 
 
 @pytest.mark.parametrize("extra", [-1, 0, 1])

@@ -32,7 +32,8 @@ def test_decode_cta_fits_beside_an_append_cta(tmp_path):
         pytest.skip(str(e))
     append = _registers("append_tc.cu", "append_tc_kernelILb0", tmp_path)  # not the self-test's form
     decode = _registers("decode.cu", "decode_kernel", tmp_path)
-    assert len(append) == 2 and len(decode) == 3, (append, decode)
+    assert len(append) == 2 and len(decode) == 5, (append, decode)
+    decode = {k: v for k, v in decode.items() if not re.search("ILi[67]E", k)}  # wide cascade items: decode steps only
     assert not any(spilled for _, spilled in [*append.values(), *decode.values()]), (append, decode)
     up = lambda regs: -(-regs // 8) * 8  # noqa: E731
     most = 3 * up(max(r for r, _ in append.values())) + up(max(r for r, _ in decode.values()))
