@@ -27,7 +27,9 @@ constexpr int kMinSharedPages = 4;    // shortest prefix worth a cascade pass
 // kernel's, and it has twice the items. The pages are still read from HBM once
 // (the subgroups' reads of a page come close together and hit L2). Measured 32
 // -> 16: 48 groups of 8 with appending rows 6341 -> 6181 us per layer (the pass
-// no longer follows the append kernel), 16 groups of 8 638 -> 610 us.
+// no longer follows the append kernel), 16 groups of 8 with two 638 -> 610 us. Over
+// fp8 pages (a pass of its own): 48 groups of 8 991 -> 985 us, 16 groups 332 -> 329.5,
+// but with own contexts of up to 300 keys 48 groups 260 -> 271.
 constexpr int kCascadeVectors = 16;
 // Where nothing runs beside the pass (calls with as many tokens as rows), items of
 // twice as many vectors (168 registers, as many CTAs: shared memory bounds them) read
@@ -41,9 +43,13 @@ constexpr int kAppendRowsMin = 64;    // smallest append tile (query rows = toke
 constexpr int kAppendTcRows = 256;    // query rows of one tcgen05 append item (two 128-row tiles)
 
 // Rows of a window of at most this many keys are not split, and the call has no
-// merge: its launch and the partials' round trip cost more than they save up to
-// 9 pages (a decode call's graph, 4 / 64 / 384 rows of 8 KV heads: 12.1 / 15.5 /
-// 27.8 us -> 10.3 / 12.2 / 26.9), but not at 17 (4 / 16 rows 13.0 / 13.7 -> 13.6 / 15.6).
+// merge, whose launch and the partials' round trip cost more than they save. KV
+// append and a decode call as a graph, 4 / 16 / 64 / 384 rows of 8 KV heads, split ->
+// not split: 128 keys 16.5 / 18.5 / 20.6 / 33.2 us -> 14.5 / 16.4 / 17.7 / 32.4, 192
+// keys 16.7 / 18.5 / 22.5 / 40.4 -> 16.5 / 18.5 / 20.5 / 39.0, 224 keys 17.0 / 18.5 /
+// 22.6 / 43.4 -> 17.7 / 18.6 / 20.6 / 42.0, 256 keys 18.5 / 18.5 / 23.6 / 47.6 -> 18.5 /
+// 20.2 / 22.5 / 45.9. Few rows gain nothing from 160 keys on and lose from 224 on:
+// the line lies below that.
 constexpr int kUnsplitWindow = 128;
 
 // Status bits, OR-ed into the first word of the workspace. They are sticky

@@ -132,10 +132,10 @@ __device__ __forceinline__ int shared_entries(const AttnParams& p, int r) {
 }
 
 // Batches of at most this many rows (one per warp of the smallest form) are
-// scanned by the planner itself, beside phase 1 in warp 0: one launch fewer
-// (5 rows of up to 65k keys 81.9 -> 81.0 us a call, 4 short rows 18.4-19.1 ->
-// 18.6). With more rows the scan is a kernel of its own, a warp per row across
-// the GPU.
+// scanned by the planner itself, a warp per row beside phase 1: one launch fewer
+// (1 / 8 short rows 18.5 / 20.5 -> 16.5 / 19.4 us as a graph, 5 rows of 20-65 thousand
+// keys 85.1 -> 84.1; eager calls 1-3 us). With more rows the scan is a kernel of its
+// own, a warp per row across the GPU.
 constexpr int kScanInPlanner = 8;
 
 // lcp[r] of every row r > 0, lcp[0] = 0.
