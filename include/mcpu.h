@@ -409,13 +409,13 @@ mcpu_status mcpu_reset_device_status(void* workspace, mcpu_stream_t stream);
  * it exercises, on a GPU and without a fault or a hang, what the tcgen05
  * append kernel does when one of its waits runs out). Runs the planner and
  * then the self-test form of that kernel as ONE CTA over the batch given
- * (same arguments and rules as mcpu_paged_attention_forward; no window, no
- * options; the batch needs an append row whose first work item spans at
- * least two 128-key blocks). In that form one role, chosen by stall_role,
+ * (same arguments and rules as mcpu_paged_attention_forward; no window, so the
+ * form for short windows is not checked, and no options; the batch needs an append
+ * row whose first work item spans at least two 128-key blocks). In that form one role, chosen by stall_role,
  * stops at the second key block of its first item and waits, for half the
  * library's wait limit, on a barrier nothing completes:
  *   0  the softmax warps of the first query tile,
- *   1  the TMA producer warp,
+ *   1  the TMA producer warp of K, the query tiles and the item queue,
  *   2  the MMA issuer of the first query tile.
  * It then raises the CTA's abort flag with its own mark (2); every other
  * role, waiting with the full limit, must leave its wait on seeing the flag

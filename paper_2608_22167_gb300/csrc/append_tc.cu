@@ -40,9 +40,9 @@
 // for a higher reference out of line, and the warp index broadcast so that what depends on it stays in
 // the uniform datapath. (Masks applied to the scores in registers also made the
 // compiler copy all 64 of them on the unmasked path.) Against the unrolled form
-// (73 KB of code, now 45): 256-row mixed batch 5300 -> 4565 us beside the
-// decode kernel, prefill of 8 prompts (35681 tokens, 1.61 TFLOP) 1677 -> 1475 us
-// = 1.09 PFLOP/s, window layer of 384 rows 250 -> 236 us. Measured slower:
+// (73 KB of code, now 45): 256-row mixed batch 5300 -> 4588 us beside the
+// decode kernel, prefill of 8 prompts (35681 tokens, 1.61 TFLOP) 1677 -> 1470 us
+// = 1.09 PFLOP/s, window layer of 384 rows 250 -> 236 us (188 with the short form). Measured slower:
 // four issuers (1737 us for the prefill), 16 softmax warps on key halves (1528),
 // 32-key chunks (1838), per-MMA elect (1556), waits in a called function (1535).
 //

@@ -54,7 +54,7 @@ def test_wait_gives_up_reports_timeout_and_leaves_the_context_usable():
 @pytest.mark.parametrize("role", [0, 1, 2], ids=["softmax", "producer", "issuer"])
 def test_append_kernel_abort_reaches_every_role(role):
     # The tcgen05 append kernel's own waits, in its self-test form: one role
-    # (softmax warps of tile A, the TMA producer, or tile A's MMA issuer)
+    # (softmax warps of tile A, the K producer, or tile A's MMA issuer)
     # stops at the second key block of its first item and waits on a barrier
     # nothing completes for half the wait limit, then raises the CTA's abort
     # flag. Every other role is then blocked on that role and waits with the
@@ -62,6 +62,8 @@ def test_append_kernel_abort_reaches_every_role(role):
     # role's mark, nobody left at the full limit), the issuers and the
     # producer drain what they had in flight, TMEM is freed, the timeout bit
     # reaches the host, and the next normal call on every SM matches the oracle.
+    # The V producer, whose waits and exit are the K producer's, is never the
+    # stalled one, and the form for short windows has no self-test of its own.
     batch = W.build_batch("abort", 91 + role, [300, 40, 700], [300, 1, 90], 16, 2)
     run = Run(batch)
     run.append()
